@@ -250,8 +250,9 @@ __global__ void __launch_bounds__(kNaThreads, 1) k_na_run(const __grid_constant_
             rs.lo = a;
             rs.hi = b;
         }
-        for (int32_t r = rs.lo + (int32_t)threadIdx.x; r < rs.hi; r += blockDim.x)
-            const_cast<NaRule*>(rs.staged)[r - rs.lo] = na_stage(na_rule(s, r));
+        // counted from 0: a rule id near INT32_MAX plus a stride would wrap
+        for (int32_t i = threadIdx.x; i < rs.hi - rs.lo; i += blockDim.x)
+            const_cast<NaRule*>(rs.staged)[i] = na_stage(na_rule(s, rs.lo + i));
     }
     const int rbytes = (int)((rs.hi - rs.lo) * (int)sizeof(NaRule));
     left -= rbytes;
@@ -263,7 +264,7 @@ __global__ void __launch_bounds__(kNaThreads, 1) k_na_run(const __grid_constant_
             e_lo = a;
             e_hi = b;
         }
-        for (int32_t e = e_lo + (int32_t)threadIdx.x; e < e_hi; e += blockDim.x) esm[e - e_lo] = s.in_src[e];
+        for (int32_t i = threadIdx.x; i < e_hi - e_lo; i += blockDim.x) esm[i] = s.in_src[e_lo + i];
     }
     for (int i = threadIdx.x; i < own; i += blockDim.x) {
         const int32_t j = lo + i;
@@ -326,20 +327,22 @@ __global__ void __launch_bounds__(kNaThreads, 1) k_na_run(const __grid_constant_
                 invalid = true;
             } else {
                 const bool staged = a >= e_lo && b <= e_hi;
-                const int32_t* const p = staged ? esm - e_lo : s.in_src;
-                // eight emissions in flight: an index out of range gives none
-                for (int32_t e = a; e < b; e += 8) {
+                const int32_t* const p = staged ? esm + (a - e_lo) : s.in_src + a;
+                // eight emissions in flight: an index out of range gives none.
+                // Counted from 0 without a sign: a list may end at INT32_MAX.
+                const uint32_t len = (uint32_t)(b - a);
+                for (uint32_t e = 0u; e < len; e += 8u) {
                     uint32_t v[8];
 #pragma unroll
-                    for (int u = 0; u < 8; ++u) {
-                        const bool there = e + u < b;
+                    for (uint32_t u = 0; u < 8u; ++u) {
+                        const bool there = e + u < len;
                         const int32_t x = there ? p[e + u] : 0;
                         const bool in = x >= 0 && x < s.q;
                         invalid |= !in;
                         v[u] = there && in ? __ldcg(Ek + x) : 0u;
                     }
 #pragma unroll
-                    for (int u = 0; u < 8; ++u) sum += (long long)v[u];
+                    for (uint32_t u = 0; u < 8u; ++u) sum += (long long)v[u];
                 }
             }
             int32_t c = Csm[i];
