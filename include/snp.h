@@ -443,7 +443,14 @@ int64_t snp_paper_format_elements(int32_t form, int64_t q, int64_t m, int64_t z)
  * All calls share the one array and the next call overwrites it (the flag
  * words are cleared at the start of every call), so calls whose work
  * overlaps on the GPU, from any thread or stream, race and must be
- * serialised by the caller.  Work is ordered on `stream`; with steps_done
+ * serialised by the caller.  All steps of a call run in one cooperative
+ * launch of up to one CTA per SM, whose CTAs meet after every step: it starts
+ * when all of them fit beside what runs on other streams, so a kernel that
+ * occupies an SM and waits for the call's result would wait for ever.  Where
+ * the device (or the partition or context in use) cannot hold that launch --
+ * no cooperative launches, or fewer than 32 SMs at the largest q -- every
+ * step is a plain launch of its own, with the same results.
+ * Work is ordered on `stream`; with steps_done
  * non-NULL the call waits for it and reports the executed step count,
  * SNP_ERR_OVERFLOW, SNP_ERR_TIMEOUT (a bounded device-side wait gave up),
  * or SNP_ERR_INVALID if the kernels found an index in the

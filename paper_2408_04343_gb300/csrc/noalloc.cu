@@ -14,7 +14,8 @@
 // keeps in shared memory as far as they fit; emissions go through L2, and the
 // CTAs meet at a counter after every step.  A launch per step spent most of
 // its time on starting and on two dependent trips to L2 per in-edge and per
-// rule field (65,537 neurons of 10 in-edges: 16.4 us per step).  Every index
+// rule field (65,537 neurons of 10 in-edges: 16.4 us per step); it remains for
+// devices that cannot hold the one launch (k_na_step).  Every index
 // read from the caller's arrays is bounds-checked, and so are the fields of
 // every rule a step fires (the ranges snp_create enforces on the host:
 // k, j, c >= 0, p and d in [0, 65535], no delay on a forgetting rule) and the
@@ -27,6 +28,7 @@
 #include <string>
 
 #include "device_common.cuh"
+#include "noalloc_plan.h"
 #include "quad.cuh"
 #include "snp_internal.h"
 
@@ -35,12 +37,13 @@ namespace snp {
 // ---- the static scratch ----------------------------------------------------
 // Layout (32-bit words): [0, 16) flag words (words 8 to 11 are the two 64-bit
 // barrier counters), [16, 24) step counters (four 64-bit values), then two
-// emission vectors of SNP_NOALLOC_MAX_Q + 1 words (the spikes sent).
+// emission vectors of SNP_NOALLOC_MAX_Q + 1 words (the spikes sent; k_na_step
+// adds the selected rule).
 constexpr int kNaFlagWords = 16;
 constexpr int kNaStepWords = 8;
 constexpr long long kNaEWords = (long long)SNP_NOALLOC_MAX_Q + 1;
 constexpr long long kNaWords = kNaFlagWords + kNaStepWords + 2 * kNaEWords;
-enum : int { kNaHalted = 3, kNaOverflow = 4, kNaInvalid = 5, kNaTimeout = 6, kNaCounters = 8 };
+enum : int { kNaAct0 = 0, kNaHalted = 3, kNaOverflow = 4, kNaInvalid = 5, kNaTimeout = 6, kNaCounters = 8 };
 enum : int { kNaBase = 0, kNaStart = 1, kNaExec = 2, kNaHalt = 3 };
 
 static __device__ __align__(256) uint32_t g_noalloc_scratch[kNaWords];
@@ -239,7 +242,7 @@ __global__ void __launch_bounds__(kNaThreads, 1) k_na_run(const __grid_constant_
     int32_t* rsm = reinterpret_cast<int32_t*>(Ssm + N);  // first rule; second half: past the last
     int32_t* osm = rsm + 2 * N;                          // list start; second half: end
     int16_t* chosen = reinterpret_cast<int16_t*>(osm + 2 * N);  // of step k at (k & 1) * N
-    const int used = (N * 28 + 15) & ~15;
+    const int used = (int)na_state_bytes(N);
     const unsigned long long base = steps[kNaBase];
     // what the CTA's first and last offsets span, when it is in range and fits
     int left = smem - used;
@@ -385,6 +388,97 @@ __global__ void __launch_bounds__(kNaThreads, 1) k_na_run(const __grid_constant_
     }
 }
 
+// One step with the state in the caller's arrays, a launch of its own: for
+// devices, partitions and contexts that cannot hold k_na_run's grid with the
+// neurons' state in shared memory (na_plan).  An emission word holds the spikes
+// sent (low 16 bits) and 1 + the local index of the selected rule.
+template <bool GATHER, bool SELECT, int SEL>
+__global__ void __launch_bounds__(256) k_na_step(NaSys s, int32_t t) {
+    uint32_t* fl = na_flags(s);
+    unsigned long long* steps = na_steps(s);
+    const unsigned long long kg = steps[kNaBase] + (unsigned long long)t;
+    const unsigned long long ks = GATHER ? kg + 1ull : kg;
+    if (GATHER) {
+        if (ld_volatile(fl + kNaHalted)) return;
+        if (ld_volatile(fl + kNaAct0 + (int)(kg % 3ull)) == 0u) {
+            if (threadIdx.x == 0) {
+                steps[kNaHalt] = kg;
+                __threadfence();
+                atomicExch(fl + kNaHalted, 1u);
+            }
+            return;
+        }
+        if (SELECT && blockIdx.x == 0 && threadIdx.x == 0) fl[kNaAct0 + (int)((kg + 2ull) % 3ull)] = 0u;
+    }
+    const int32_t j = (int32_t)(blockIdx.x * blockDim.x + threadIdx.x);
+    bool active = false;
+    if (j < s.q) {
+        int32_t r0 = s.rule_off[j], r1 = s.rule_off[j + 1];
+        int32_t c = s.C[j];
+        bool ok = r0 >= 0 && r0 <= r1 && (long long)r1 <= s.m && r1 - r0 <= kMaxRulesPerNeuron && c >= 0;
+        const int32_t P = s.P[j], D = s.D[j];
+        uint32_t st = 0u;
+        if (P != -1) {
+            ok = ok && P >= r0 && P < r1 && D >= 0 && D <= (int32_t)kDMask;
+            st = ((uint32_t)(P - r0 + 1) << kPendShift) | ((uint32_t)D & kDMask);
+        } else {
+            ok = ok && D == 0;  // a neuron can only be closed by a pending rule
+        }
+        if (!ok) {
+            atomicOr(fl + kNaInvalid, 1u);
+            r0 = r1 = 0;
+            st = 0u;
+        }
+        if (GATHER) {
+            const uint32_t* Ek = na_e(s, kg);
+            const int32_t a = s.in_off[j], b = s.in_off[j + 1];
+            long long sum = 0;
+            if (a < 0 || a > b || (long long)b > s.nin) {
+                atomicOr(fl + kNaInvalid, 1u);
+            } else {
+                for (int32_t e = a; e < b; ++e) {
+                    const int32_t src = s.in_src[e];
+                    if (src < 0 || src >= s.q) {
+                        atomicOr(fl + kNaInvalid, 1u);
+                        continue;
+                    }
+                    sum += (long long)(Ek[src] & 0xffffu);
+                }
+            }
+            if ((st >> kPendShift) == 0u) {
+                long long nc = (long long)c + sum;
+                if (nc > 2147483647ll) {
+                    atomicOr(fl + kNaOverflow, 1u);
+                    nc = 2147483647ll;
+                }
+                c = (int32_t)nc;
+            }
+            // step kg is executed: publish its spiking vector
+            const uint32_t sel = Ek[j] >> 16;
+            s.S[j] = sel ? r0 + (int32_t)sel - 1 : -1;
+        }
+        if (SELECT) {
+            const NaRules none{nullptr, 0, 0};
+            bool bad = false;
+            const SelOut o = na_select<SEL>(s, none, j, r0, r1, c, st, ks, &bad);
+            if (bad) atomicOr(fl + kNaInvalid, 1u);
+            c = o.c_after;
+            active = o.active;
+            na_e(s, ks)[j] = ((uint32_t)o.emit & 0xffffu) | ((uint32_t)(o.s + 1) << 16);
+            const uint32_t pend = o.st >> kPendShift;
+            s.P[j] = pend ? r0 + (int32_t)pend - 1 : -1;
+            s.D[j] = pend ? (int32_t)(o.st & kDMask) : 0;
+        }
+        s.C[j] = c;
+    }
+    if (SELECT) {
+        if (__syncthreads_or(active) && threadIdx.x == 0) {
+            uint32_t* a = fl + kNaAct0 + (int)(ks % 3ull);
+            if (ld_volatile(a) == 0u) atomicExch(a, 1u);
+        }
+    }
+}
+
 // Clears the flags and sets the base step (first), or clears the barrier
 // counters for a further launch of the call.
 __global__ void k_na_begin(NaSys s, unsigned long long k0, int first) {
@@ -397,6 +491,26 @@ __global__ void k_na_begin(NaSys s, unsigned long long k0, int first) {
         st[kNaExec] = 0ull;
         st[kNaHalt] = 0ull;
     }
+}
+
+__global__ void k_na_finish(NaSys s, int32_t tail) {
+    if (threadIdx.x == 0 && blockIdx.x == 0) {
+        unsigned long long* st = na_steps(s);
+        if (ld_volatile(na_flags(s) + kNaHalted))
+            st[kNaBase] = st[kNaHalt];
+        else
+            st[kNaBase] += (unsigned long long)tail;
+        st[kNaExec] = st[kNaBase] - st[kNaStart];
+    }
+}
+
+template <bool G, bool S>
+static void na_launch(const NaSys& s, int32_t t, int sel, cudaStream_t st) {
+    const unsigned grid = (unsigned)((s.q + 255) / 256);
+    if (sel == SNP_SELECT_FIRST)
+        k_na_step<G, S, SNP_SELECT_FIRST><<<grid, 256, 0, st>>>(s, t);
+    else
+        k_na_step<G, S, SNP_SELECT_PHILOX><<<grid, 256, 0, st>>>(s, t);
 }
 
 // Device address of the scratch array, looked up once per device.  The
@@ -425,12 +539,47 @@ static int na_scratch(uint32_t** out) {
     return SNP_OK;
 }
 
+// All steps by k_na_run.
+static cudaError_t na_run(const NaSys& s, const NaPlan& pl, int cap, int select, uint64_t step, int64_t n,
+                          cudaStream_t st) {
+    auto fn = select == SNP_SELECT_FIRST ? k_na_run<SNP_SELECT_FIRST> : k_na_run<SNP_SELECT_PHILOX>;
+    // the same bound for every launch: threads may launch different sizes at once
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, cap - 1024);
+    for (int64_t done = 0; done < n && e == cudaSuccess; done += kNaMaxSteps) {
+        k_na_begin<<<1, 32, 0, st>>>(s, (unsigned long long)step, done == 0 ? 1 : 0);
+        if ((e = cudaGetLastError()) != cudaSuccess) break;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)pl.G);
+        cfg.blockDim = dim3(kNaThreads);
+        cfg.dynamicSmemBytes = (size_t)pl.smem;
+        cfg.stream = st;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeCooperative;
+        at[0].val.cooperative = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        e = cudaLaunchKernelEx(&cfg, fn, s, (long long)std::min<int64_t>(n - done, kNaMaxSteps), pl.N, pl.smem,
+                               done > 0 ? 1 : 0);
+    }
+    return e;
+}
+
+// All steps by a launch of k_na_step each.
+static cudaError_t na_run_steps(const NaSys& s, int select, uint64_t step, int64_t n, cudaStream_t st) {
+    k_na_begin<<<1, 32, 0, st>>>(s, (unsigned long long)step, 1);
+    na_launch<false, true>(s, 0, select, st);
+    for (int64_t t = 0; t + 1 < n; ++t) na_launch<true, true>(s, (int32_t)t, select, st);
+    na_launch<true, false>(s, (int32_t)(n - 1), select, st);
+    k_na_finish<<<1, 32, 0, st>>>(s, (int32_t)n);
+    return cudaGetLastError();
+}
+
 }  // namespace snp
 
 using namespace snp;
 
-extern "C" int snp_step_noalloc(const snp_device_system* d, int32_t select, uint64_t seed, uint64_t step, int64_t n,
-                                void* stream, int64_t* steps_done) {
+extern "C" int snp_noalloc_on(const snp_device_system* d, int32_t select, uint64_t seed, uint64_t step, int64_t n,
+                              void* stream, int64_t* steps_done, int32_t sms, int32_t cap) {
     if (steps_done) *steps_done = 0;
     if (!d) return fail(SNP_ERR_INVALID, "system is NULL");
     if (d->q < 1 || d->q > SNP_NOALLOC_MAX_Q)
@@ -465,36 +614,14 @@ extern "C" int snp_step_noalloc(const snp_device_system* d, int32_t select, uint
     s.scratch = scratch;
     s.seed = seed;
     cudaStream_t st = (cudaStream_t)stream;
-    // 128 neurons per CTA at least (fewer CTAs meet sooner), one CTA per SM at most
-    int dev = 0, sms = 0, cap = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&cap, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess || sms < 1)
-        return fail(SNP_ERR_CUDA, "snp_step_noalloc: device query");
-    const int N = std::max(128, (int)((s.q + sms - 1) / sms));
-    const int G = (int)((s.q + N - 1) / N);
-    // per neuron 28 bytes and, of its rules and in-neighbours, what 1 KB holds
-    const int smem = (int)std::min<long long>(cap - 1024, (long long)N * 1024);
-    auto fn = select == SNP_SELECT_FIRST ? k_na_run<SNP_SELECT_FIRST> : k_na_run<SNP_SELECT_PHILOX>;
-    // the same bound for every launch: threads may launch different sizes at once
-    cudaError_t le = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, cap - 1024);
-    for (int64_t done = 0; done < n && le == cudaSuccess; done += kNaMaxSteps) {
-        k_na_begin<<<1, 32, 0, st>>>(s, (unsigned long long)step, done == 0 ? 1 : 0);
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)G);
-        cfg.blockDim = dim3(kNaThreads);
-        cfg.dynamicSmemBytes = (size_t)smem;
-        cfg.stream = st;
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeCooperative;
-        at[0].val.cooperative = 1;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
-        le = cudaLaunchKernelEx(&cfg, fn, s, (long long)std::min<int64_t>(n - done, kNaMaxSteps), N, smem, done > 0 ? 1 : 0);
+    const NaPlan pl = na_plan(d->q, sms, cap);
+    cudaError_t le = pl.G > 0 ? na_run(s, pl, cap, select, step, n, st) : cudaErrorCooperativeLaunchTooLarge;
+    if (le == cudaErrorCooperativeLaunchTooLarge) {  // the state, or the grid, does not fit at once
+        cudaGetLastError();
+        le = na_run_steps(s, select, step, n, st);
     }
     if (le != cudaSuccess) cudaGetLastError();
     if (le != cudaSuccess) return fail(SNP_ERR_CUDA, std::string("snp_step_noalloc launch: ") + cudaGetErrorString(le));
-    if (cudaGetLastError() != cudaSuccess) return fail(SNP_ERR_CUDA, "snp_step_noalloc launch failed");
     if (!steps_done) return SNP_OK;
     uint32_t fl[kNaFlagWords];
     unsigned long long sw[4];
@@ -509,4 +636,17 @@ extern "C" int snp_step_noalloc(const snp_device_system* d, int32_t select, uint
     if (fl[kNaInvalid]) return fail(SNP_ERR_INVALID, "an index or a fired rule's field in the device arrays was out of range");
     if (fl[kNaOverflow]) return fail(SNP_ERR_OVERFLOW, "a spike count left the int32 range");
     return SNP_OK;
+}
+
+extern "C" int snp_step_noalloc(const snp_device_system* d, int32_t select, uint64_t seed, uint64_t step, int64_t n,
+                                void* stream, int64_t* steps_done) {
+    int dev = 0, sms = 0, cap = 0, coop = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&cap, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess) {
+        cudaGetLastError();
+        sms = cap = coop = 0;  // the arguments are checked before the device
+    }
+    return snp_noalloc_on(d, select, seed, step, n, stream, steps_done, coop ? sms : 0, cap);
 }

@@ -2,11 +2,14 @@
 at entry INT32_MAX and rules at the last id, where an index plus a stride no
 longer fits 32 bits.  State and executed steps equal the oracle's.
 """
+import ctypes as ct
+
 import numpy as np
 import pytest
 
 import oracle
 from paper_2408_04343_gb300 import libsnp, synth
+from test_zz_no_alloc import device_tables, fresh_state
 
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
@@ -56,3 +59,40 @@ def test_lists_and_rules_at_the_ends_of_the_largest_arrays(q):
     assert (C.cpu().numpy() == st[0]).all() and (D.cpu().numpy() == 0).all() and (P.cpu().numpy() == -1).all()
     if ex:
         assert (S.cpu().numpy() == np.where(S_ref >= 0, S_ref + (m - q), -1)).all()
+
+
+def call_on(sms, cap, d, tabs, C, D, P, S, select, seed, step, n):
+    """snp_step_noalloc as on a device of sms SMs with cap bytes of shared memory."""
+    fn = libsnp.load().snp_noalloc_on
+    p = lambda t: t.data_ptr()
+    s = libsnp.snp_device_system(d.q, d.m, tabs["in_sources"].numel(), *(p(tabs[k]) for k in (
+        "rule_offsets", "rule_k", "rule_j", "rule_c", "rule_p", "rule_d", "in_offsets", "in_sources")),
+        p(C), p(D), p(P), p(S))
+    done = ct.c_int64(0)
+    rc = fn(ct.byref(s), ct.c_int32(select), ct.c_uint64(seed), ct.c_uint64(step), ct.c_int64(n), None,
+            ct.byref(done), ct.c_int32(sms), ct.c_int32(cap))
+    return rc, int(done.value)
+
+
+# (SMs, shared memory): no cooperative launches; 18 SMs cannot hold 200,000
+# neurons' state; 100 KB hold 4 SMs' share of 9,000; few rules and lists staged
+@pytest.mark.parametrize("q,sms,cap", [(9000, 0, 0), (200_000, 18, 232448), (9000, 4, 102400), (9000, 3, 102400),
+                                       (3000, 9, 14_000), (1, 1, 232448)])
+@pytest.mark.parametrize("mode", [oracle.FIRST, oracle.PHILOX])
+def test_devices_that_hold_less(q, sms, cap, mode):
+    d = synth.random_system(q, 70 + q, outdeg=(min(2, q - 1), min(9, q - 1)), rules=(2, 6), d_range=(0, 3),
+                            spikes=(0, 10))
+    tabs = device_tables(d)
+    C, D, P, S = fresh_state(d)
+    st, k = oracle.initial_state(d), 0
+    select = libsnp.SNP_SELECT_FIRST if mode == oracle.FIRST else libsnp.SNP_SELECT_PHILOX
+    for n in (1, 7, 40):
+        rc, done = call_on(sms, cap, d, tabs, C, D, P, S, select, 11, k, n)
+        ex, S_ref = oracle.run(d, st, n, mode, 11, step0=k)
+        assert rc == 0 and done == ex
+        k += ex
+        assert (C.cpu().numpy() == st[0]).all() and (D.cpu().numpy() == st[1]).all()
+        assert (P.cpu().numpy() == st[2]).all()
+        assert not ex or (S.cpu().numpy() == S_ref).all()
+    C[q // 2] = -1  # checked on every form
+    assert call_on(sms, cap, d, tabs, C, D, P, S, select, 11, k, 2)[0] == libsnp.SNP_ERR_INVALID
