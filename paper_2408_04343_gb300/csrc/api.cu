@@ -12,6 +12,7 @@
 
 #include "kernels.h"
 #include "snp_internal.h"
+#include "pointer_kind.h"
 #include "system.h"
 
 namespace snp {
@@ -244,7 +245,18 @@ bool is_device_ptr(const void* p) {
         cudaGetLastError();
         return false;
     }
-    return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
+    return is_device_memory(a);
+}
+
+// Memory that a kernel on the current device may read in place.
+static bool in_place_ptr(const void* p) {
+    cudaPointerAttributes a;
+    int dev = 0;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return readable_in_place(a, dev);
 }
 
 // ---- chunk graphs of the grid-wide engines ------------------------------
@@ -1150,8 +1162,8 @@ int snp_get_state(const snp_system* s, int32_t* C, int32_t* D, int32_t* P, int64
     return SNP_OK;
 }
 
-// Imports (C, D, P) on the device: arrays in device memory are read where they
-// are, others are copied into buffers whose contents set_state discards anyway
+// Imports (C, D, P) on the device: arrays in this device's memory are read where
+// they are, others (host memory, another GPU's) are copied into buffers whose contents set_state discards anyway
 // (the spiking vectors and the export scratch).  One launch checks, a second
 // writes in slot order if every neuron passed, and the host waits once for the
 // verdict.
@@ -1162,8 +1174,8 @@ int snp_set_state(snp_system* s, const int32_t* C, const int32_t* D, const int32
     if (len < s->q) return fail(SNP_ERR_INVALID, "state shorter than q");
     cudaStream_t st = s->stream;
     const size_t bytes = sizeof(int32_t) * (size_t)s->q;
-    const bool direct = ((uintptr_t)C | (uintptr_t)D | (uintptr_t)P) % sizeof(int32_t) == 0 && is_device_ptr(C) &&
-                        is_device_ptr(D) && is_device_ptr(P);
+    const bool direct = ((uintptr_t)C | (uintptr_t)D | (uintptr_t)P) % sizeof(int32_t) == 0 && in_place_ptr(C) &&
+                        in_place_ptr(D) && in_place_ptr(P);
     const int32_t *sc = C, *sd = D, *sp = P;
     if (!direct) {
         if (cudaMemcpyAsync(s->scratch, C, bytes, cudaMemcpyDefault, st) != cudaSuccess ||
