@@ -1163,10 +1163,11 @@ int snp_get_state(const snp_system* s, int32_t* C, int32_t* D, int32_t* P, int64
 }
 
 // Imports (C, D, P) on the device: arrays in this device's memory are read where
-// they are, others (host memory, another GPU's) are copied into buffers whose contents set_state discards anyway
-// (the spiking vectors and the export scratch).  One launch checks, a second
-// writes in slot order if every neuron passed, and the host waits once for the
-// verdict.
+// they are (once: other streams may still write them), others (host memory,
+// another GPU's) are copied, both into buffers whose contents set_state discards
+// anyway (the spiking vectors and the export scratch).  One launch checks, a
+// second writes in slot order if every neuron passed, and the host waits once
+// for the verdict.
 int snp_set_state(snp_system* s, const int32_t* C, const int32_t* D, const int32_t* P, int64_t len, uint64_t step) {
     if (!s || !C || !D || !P) return fail(SNP_ERR_INVALID, "NULL argument");
     if (s->busy.load()) return fail(SNP_ERR_BUSY, "system is owned by an unfinished batch");
@@ -1188,9 +1189,10 @@ int snp_set_state(snp_system* s, const int32_t* C, const int32_t* D, const int32
     }
     uint32_t bad = 0xffffffffu;
     if (cudaMemsetAsync(s->dev.flags + kFlagImport, 0xff, sizeof(uint32_t), st) != cudaSuccess ||
-        launch_import(s->dev, s->d_rule_base, sc, sd, sp, step, direct, st) != cudaSuccess)
+        launch_import(s->dev, s->d_rule_base, sc, sd, sp, step, direct ? s->scratch : nullptr, st) != cudaSuccess)
         return cuda_fail("state import");
-    // the spiking vectors held the staged D and P: all -1 again either way
+    // the spiking vectors held the staged D and P: all -1 again either way (in
+    // place, the commit has done that)
     if (!direct && (cudaMemsetAsync(s->dev.S[0], 0xff, bytes, st) != cudaSuccess ||
                     cudaMemsetAsync(s->dev.S[1], 0xff, bytes, st) != cudaSuccess))
         return cuda_fail("state upload");

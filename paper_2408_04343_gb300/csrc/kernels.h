@@ -25,10 +25,11 @@ cudaError_t launch_export(const DevSys& s, const int32_t* rule_base, int what, i
 // device.  The check records the smallest neuron id whose values are out of
 // range in flags[kFlagImport] (which the caller sets to 0xffffffff first); the
 // commit, if there is none, writes C and the status words in slot order, the
-// step words and flags, and (spiking: C, D and P are not staged there) the
-// spiking vectors.
+// step words and flags.  hold (q words): C, D and P are the caller's arrays; what
+// the check read of them is kept there and in the spiking vectors, and is what
+// the commit writes.  NULL: they are private copies, read by both launches.
 cudaError_t launch_import(const DevSys& s, const int32_t* rule_base, const int32_t* C, const int32_t* D,
-                          const int32_t* P, unsigned long long step, bool spiking, cudaStream_t st);
+                          const int32_t* P, unsigned long long step, int32_t* hold, cudaStream_t st);
 
 // CTA-resident engine (kernels_resident.cu): each CTA takes whole systems
 // from `work` (largest first as listed) and runs all their steps.

@@ -294,13 +294,17 @@ __global__ void k_export(const DevSys s, const int32_t* __restrict__ rule_base, 
 // State import: the caller's C, D, P (neuron order, on the device) checked
 // neuron by neuron with the ranges snp_set_state documents, then, only if all
 // passed (flags[kFlagImport] untouched), written in slot order (spikes, and the
-// status word: 1 + local pending rule above D) with the step words, cleared
-// flags and (spiking) the spiking vectors at -1.  Both launches go out at once:
-// the second reads the first one's verdict, so the host waits once.
+// status word: 1 + local pending rule above D) with the step words and cleared
+// flags.  Both launches go out at once: the second reads the first one's
+// verdict, so the host waits once.
+// hold: C, D and P are the caller's own arrays, which another stream may still
+// write.  Each value is then read once: the check keeps what it read, in slot
+// order, in hold and the spiking vectors; the commit writes that and leaves the
+// spiking vectors at -1.
 template <bool COMMIT>
 __global__ void k_import(DevSys s, const int32_t* __restrict__ rule_base, const int32_t* __restrict__ C,
                          const int32_t* __restrict__ D, const int32_t* __restrict__ P, unsigned long long step,
-                         int spiking) {
+                         int32_t* hold) {
     const int32_t slot = blockIdx.x * blockDim.x + threadIdx.x;
     if (COMMIT) {
         if (__ldcg(s.flags + kFlagImport) != 0xffffffffu) return;
@@ -315,7 +319,10 @@ __global__ void k_import(DevSys s, const int32_t* __restrict__ rule_base, const 
     }
     if (slot >= s.q) return;
     const uint32_t i = neuron_id(s, slot);
-    const int32_t c = C[i], d = D[i], p = P[i];
+    const bool held = COMMIT && hold != nullptr;
+    const int32_t c = held ? hold[slot] : *(const volatile int32_t*)(C + i);
+    const int32_t d = held ? s.S[0][slot] : *(const volatile int32_t*)(D + i);
+    const int32_t p = held ? s.S[1][slot] : *(const volatile int32_t*)(P + i);
     const int32_t r0 = rule_base[slot];
     if (!COMMIT) {
         bool ok = c >= 0 && d >= 0 && d <= kMaxDelay;
@@ -324,22 +331,27 @@ __global__ void k_import(DevSys s, const int32_t* __restrict__ rule_base, const 
         else
             ok = ok && p >= r0 && p - r0 < rule_hi(s, slot) - rule_lo(s, slot);
         if (!ok) atomicMin(s.flags + kFlagImport, i);
+        if (hold) {
+            hold[slot] = c;
+            s.S[0][slot] = d;
+            s.S[1][slot] = p;
+        }
         return;
     }
     s.C[slot] = c;
     s.st[slot] = p == -1 ? 0u : ((uint32_t)(p - r0 + 1) << kPendShift) | (uint32_t)d;
-    if (spiking) {
+    if (held) {
         s.S[0][slot] = -1;
         s.S[1][slot] = -1;
     }
 }
 
 cudaError_t launch_import(const DevSys& s, const int32_t* rule_base, const int32_t* C, const int32_t* D,
-                          const int32_t* P, unsigned long long step, bool spiking, cudaStream_t st) {
+                          const int32_t* P, unsigned long long step, int32_t* hold, cudaStream_t st) {
     if (s.q == 0) return cudaSuccess;
     const unsigned grid = (unsigned)((s.q + 255) / 256);
-    k_import<false><<<grid, 256, 0, st>>>(s, rule_base, C, D, P, step, 0);
-    k_import<true><<<grid, 256, 0, st>>>(s, rule_base, C, D, P, step, spiking ? 1 : 0);
+    k_import<false><<<grid, 256, 0, st>>>(s, rule_base, C, D, P, step, hold);
+    k_import<true><<<grid, 256, 0, st>>>(s, rule_base, C, D, P, step, hold);
     return cudaGetLastError();
 }
 
