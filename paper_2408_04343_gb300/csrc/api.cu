@@ -1,4 +1,5 @@
 // C-ABI of libsnp: system life cycle, stepping, state access.
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -550,26 +551,61 @@ static int step_ell_forms(snp_system* s, int64_t n) {
     return SNP_OK;
 }
 
-// Page-locked bytes for small reads back, one piece per thread for as long as
-// it lives: a copy into pageable memory is staged by the driver, about 5 us
-// each time.  NULL when there are none to be had.
+// Id of the current context, unique for the life of the process (0: unknown):
+// after cudaDeviceReset the same device has another one.
+static unsigned long long context_id() {
+    using Fn = CUresult (*)(CUcontext, unsigned long long*);
+    static const Fn fn = [] {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &p, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            p = nullptr;
+        }
+        return reinterpret_cast<Fn>(p);
+    }();
+    unsigned long long id = 0;
+    return fn && fn(nullptr, &id) == CUDA_SUCCESS ? id : 0;
+}
+
+// Page-locked bytes for small reads back, one piece per thread and context for
+// as long as both live: a copy into pageable memory is staged by the driver,
+// about 5 us each time (a piece per system would cost its creation 100 us and
+// its end 155).  NULL when there are none to be had.
 struct PinnedWords {
-    void* p = nullptr;
-    bool tried = false;
+    static constexpr int kContexts = 4;  // of one thread; beyond them, pageable copies
+    unsigned long long ctx[kContexts] = {};
+    void* p[kContexts] = {};
     ~PinnedWords() {
-        if (p && cudaFreeHost(p) != cudaSuccess) cudaGetLastError();  // the context may be gone
+        // Only the current context's piece is known to exist still.  In the
+        // relaxed capture mode: in the default one the call would fail, and
+        // spoil the capture, while another thread captures a stream.
+        const unsigned long long id = context_id();
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        for (int i = 0; i < kContexts && id != 0; ++i)
+            if (ctx[i] == id && p[i]) {
+                cudaThreadExchangeStreamCaptureMode(&mode);
+                if (cudaFreeHost(p[i]) != cudaSuccess) cudaGetLastError();
+                cudaThreadExchangeStreamCaptureMode(&mode);
+            }
     }
 };
 static void* pinned_words() {
     static thread_local PinnedWords w;
-    if (!w.tried) {
-        w.tried = true;
-        if (cudaHostAlloc(&w.p, kStatusBytes, cudaHostAllocPortable) != cudaSuccess) {
+    const unsigned long long id = context_id();
+    if (id == 0) return nullptr;
+    for (int i = 0; i < PinnedWords::kContexts; ++i) {
+        if (w.ctx[i] == id) return w.p[i];
+        if (w.ctx[i] != 0) continue;
+        w.ctx[i] = id;  // asked for once, whatever comes of it
+        if (cudaHostAlloc(&w.p[i], kStatusBytes, cudaHostAllocDefault) != cudaSuccess) {
             cudaGetLastError();
-            w.p = nullptr;
+            w.p[i] = nullptr;
         }
+        return w.p[i];
     }
-    return w.p;
+    return nullptr;
 }
 
 // Copies `bytes` (at most kStatusBytes) from the device and waits.
