@@ -441,9 +441,10 @@ static int step_grid(snp_system* s, int64_t n) {
     return SNP_OK;
 }
 
-// The grid-resident launch of an AUTO system in quad order; false when the
-// packed emissions and the state of a CTA's groups do not fit, or the device
-// cannot hold the grid at once.
+// The grid-resident launch of an AUTO system in quad order (hp.quad_ptr32 given);
+// false when the packed emissions and the state of a CTA's groups do not fit,
+// the device cannot hold the grid at once, or a long in-list would keep one
+// warp busy.
 static bool grid_plan(snp_system* s, const HostPack& hp, int sms) {
     GridSys& gs = s->grid;
     const int ng = (hp.q + kGroup - 1) / kGroup;
@@ -459,7 +460,7 @@ static bool grid_plan(snp_system* s, const HostPack& hp, int sms) {
     int64_t most = 0;
     for (int r = 0; r < gs.G; ++r) {
         int64_t cols = 0;
-        for (int g = r; g < ng; g += gs.G) cols += ptr.empty() ? 0 : ptr[(size_t)g + 1] - ptr[(size_t)g];
+        for (int g = r; g < ng; g += gs.G) cols += ptr[(size_t)g + 1] - ptr[(size_t)g];
         most = std::max(most, cols);
     }
     // several warps per group as in cluster_plan: one for every 16 columns
@@ -482,7 +483,7 @@ static bool grid_plan(snp_system* s, const HostPack& hp, int sms) {
     const size_t cap = (size_t)resident_max_smem() - 1024;
     const int cols = (int)std::min<int64_t>(most, 1 << 20);
     gs.rules = (int32_t)rules;
-    gs.lsm = !ptr.empty();
+    gs.lsm = 1;
     size_t b = grid_smem_bytes(gs.mode, gs, gs.lsm, cols, gs.rules);
     if (b > cap && gs.rules > 0) {
         gs.rules = 0;
@@ -495,7 +496,23 @@ static bool grid_plan(snp_system* s, const HostPack& hp, int sms) {
         if (b > cap) b = grid_smem_bytes(gs.mode, gs, false, 0, gs.rules = 0);
     }
     gs.smem = (int32_t)b;
-    return b <= cap;
+    if (b > cap) return false;
+    // A group's lists are as long as its longest one, and a few warps of one CTA
+    // walk them, where the tiled engine deals all in-edges evenly to the chip's
+    // threads.  From L2 a column costs a warp some 0.03 us (from shared memory a
+    // third, and what fits there is short).  Without long lists a tiled step
+    // takes 4 us more than a grid-resident one with compiled records, 6 at
+    // 400,000 neurons, 12 to 15 more with test records or rule tables, 2 more
+    // with the rule table itself.  us per step, grid / tiled, one neuron of 250,
+    // 500, 1,000, 2,000 in-edges among neurons of 10: 32,768 neurons 4.0, 5.6, 7.9,
+    // 12.5 / 7.1; 200,000 neurons 11.3, 18.8, 33, 62 / 8.6; 100,000 neurons with
+    // test records 9.6, 13.4, 21, 37 / 17.4; 60,000 with rule tables 7.6, 10, 13.7,
+    // 21.2 / 21.1.  100,000 neurons of power-law in-degrees (rank^-0.8, longest
+    // list 19,745): 295 / 8.2.
+    const int warps = gs.threads / 32;
+    const int64_t even = hp.nsyn / ((int64_t)kGroup * gs.G * warps);
+    const int spare = gs.mode == kClusterTest8 || gs.mode == kClusterTable ? 352 : 96;
+    return gs.lsm || grid_longest_walk(ptr, gs.G, warps, S) - even <= spare + hp.q / 8192;
 }
 
 // Which layouts a system needs, from its options and size (before packing).
@@ -835,12 +852,17 @@ int snp_create(const snp_desc* desc, const snp_options* opts, snp_system** out) 
     // rule table itself
     if (hp.quads && !s->compiled && !(s->tables = build_rule_tables(desc, &hp)))
         s->test_recs = build_test_records(desc, &hp);
-    if (want_tiled && hp.quads && (int64_t)hp.max_in * (int64_t)hp.max_p <= (int64_t)INT32_MAX && grid_plan(s, hp, sms)) {
-        pack_in_quads32(desc, &hp, s->grid.e_bits);
+    if (want_tiled && hp.quads && (int64_t)hp.max_in * (int64_t)hp.max_p <= (int64_t)INT32_MAX) {
+        quad_list_starts(hp, 1, &hp.quad_ptr32);
         s->has_grid = grid_plan(s, hp, sms);
-        want_in = hp.q <= kMaxQuadQ;  // for batches
+        if (s->has_grid) {
+            pack_in_quads32(desc, &hp, s->grid.e_bits);
+            want_in = hp.q <= kMaxQuadQ;  // for batches
+        }
     }
-    if (want_tiled && !s->has_grid && grid_size) {  // not for its size: the caller's order for the tiled engine
+    // not so after all: the caller's order for the tiled engine, unless batches
+    // want the quads
+    if (want_tiled && !s->has_grid && hp.quads && hp.q > kBatchResidentMaxQ) {
         hp = HostPack();
         s->tables = s->test_recs = false;
         window = 0;
@@ -879,7 +901,8 @@ int snp_create(const snp_desc* desc, const snp_options* opts, snp_system** out) 
             s->has_tiled = true;
             // the resident engine (batches) still needs in-lists when the system fits one CTA
             if (o.engine == SNP_ENGINE_AUTO)
-                want_in = resident_smem_bytes(hp.q, resident_e_bits(hp.max_p)) + 1024 <= (size_t)optin;
+                want_in = hp.q <= kBatchResidentMaxQ &&
+                          resident_smem_bytes(hp.q, resident_e_bits(hp.max_p)) + 1024 <= (size_t)optin;
         } else if (o.engine == SNP_ENGINE_TILED) {
             delete s;
             return st;

@@ -124,7 +124,6 @@ struct Autotune {
         fclose(f);
     }
 };
-constexpr int kBatchResidentMaxQ = 65536;    // larger systems run grid-wide
 
 }  // namespace snp
 

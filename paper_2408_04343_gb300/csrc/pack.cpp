@@ -116,6 +116,28 @@ void pack_in_lists(const snp_desc* d, HostPack* hp) {
     }
 }
 
+void quad_list_starts(const HostPack& hp, int per, std::vector<int32_t>* ptr) {
+    const int32_t ng = (hp.q + kGroup - 1) / kGroup;
+    ptr->assign((size_t)ng + 1, 0);
+    for (int32_t g = 0; g < ng; ++g) {
+        int32_t w = 0;
+        for (int32_t s = g * kGroup; s < std::min(hp.q, (g + 1) * kGroup); ++s) w = std::max(w, hp.indeg[(size_t)hp.perm[s]]);
+        (*ptr)[g + 1] = (*ptr)[g] + (w + per - 1) / per;
+    }
+}
+
+int32_t grid_longest_walk(const std::vector<int32_t>& ptr, int G, int warps, int warps_per_group) {
+    const int ng = (int)ptr.size() - 1, nw = std::max(1, warps / warps_per_group);
+    std::vector<int32_t> walk((size_t)G * nw, 0);
+    int32_t most = 0;
+    for (int g = 0; g < ng; ++g) {  // group g is the g / G-th of CTA g mod G
+        int32_t& w = walk[(size_t)(g % G) * nw + (size_t)(g / G) % nw];
+        w += (ptr[(size_t)g + 1] - ptr[(size_t)g] + warps_per_group - 1) / warps_per_group;
+        most = std::max(most, w);
+    }
+    return most;
+}
+
 // The columns of a quad-order system's in-lists, `per` sources of each neuron
 // per column: ptr gets the groups' first columns, alloc(columns) makes room
 // for them, put(column, lane, j, h, place) stores source h of the lane's j-th
@@ -147,12 +169,7 @@ static void quad_columns(const snp_desc* d, const HostPack* hp, int per, std::ve
             for (int64_t e = d->syn_offsets[i]; e < d->syn_offsets[i + 1]; ++e)
                 src[(size_t)fill[(size_t)place[(size_t)d->syn_targets[e]]]++] = place[(size_t)i];
     }
-    ptr->assign((size_t)ng + 1, 0);
-    for (int32_t g = 0; g < ng; ++g) {
-        int32_t w = 0;
-        for (size_t x = (size_t)g * kGroup; x < (size_t)(g + 1) * kGroup; ++x) w = std::max(w, off[x + 1] - off[x]);
-        (*ptr)[g + 1] = (*ptr)[g] + (w + per - 1) / per;
-    }
+    quad_list_starts(*hp, per, ptr);
     alloc((size_t)(*ptr)[ng]);
     for (int32_t g = 0; g < ng; ++g) {
         const int32_t w = ((*ptr)[g + 1] - (*ptr)[g]) * per;
@@ -250,7 +267,8 @@ int pack_system(const snp_desc* d, bool want_out_lists, bool want_in_lists, int 
     if (sort_slots && window < kSlice) window = kSlice;
 
     // in-degrees
-    std::vector<int32_t> indeg(q, 0);
+    std::vector<int32_t>& indeg = hp->indeg;
+    indeg.assign((size_t)q, 0);
     for (int64_t e = 0; e < nsyn; ++e) indeg[d->syn_targets[e]]++;
     hp->max_in = q ? *std::max_element(indeg.begin(), indeg.end()) : 0;
     hp->max_out = 0;

@@ -105,6 +105,7 @@ struct HostPack {
     bool identity = false;      // slot order == caller's order
     bool quads = false;         // slots in groups of quads (see pack_system)
     bool compact = true;
+    std::vector<int32_t> indeg;       // [q] in-degrees, by neuron
     std::vector<int32_t> perm;        // slot -> neuron
     std::vector<int32_t> inv;         // neuron -> slot
     std::vector<int32_t> rule_off;    // [q+1] slot order
@@ -312,6 +313,12 @@ void pack_in_quads(const snp_desc* d, HostPack* hp);
 // one source of each of a lane's neurons per column, (byte address of the
 // source's word in the packed vector) << 8 | its first bit in the word.
 void pack_in_quads32(const snp_desc* d, HostPack* hp, int eb);
+// First columns of the groups' in-lists at `per` sources of each neuron per column.
+void quad_list_starts(const HostPack& hp, int per, std::vector<int32_t>* ptr);
+// Most columns one warp of the grid-resident engine walks: G CTAs of `warps`
+// warps, group g on CTA g mod G, there on one warp in turn or split over
+// warps_per_group of them.
+int32_t grid_longest_walk(const std::vector<int32_t>& ptr, int G, int warps, int warps_per_group);
 // Slot of the j-th neuron of quad `lane` of group g in a system of q neurons,
 // -1 past its end.  The last group may be partial: its quads' first neurons
 // still come first, without gaps.
