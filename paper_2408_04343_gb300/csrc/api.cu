@@ -857,7 +857,7 @@ int snp_create(const snp_desc* desc, const snp_options* opts, snp_system** out) 
         s->has_grid = grid_plan(s, hp, sms);
         if (s->has_grid) {
             pack_in_quads32(desc, &hp, s->grid.e_bits);
-            want_in = hp.q <= kMaxQuadQ;  // for batches
+            want_in = hp.q <= kBatchResidentMaxQ;  // for batches
         }
     }
     // not so after all: the caller's order for the tiled engine, unless batches
@@ -926,11 +926,15 @@ int snp_create(const snp_desc* desc, const snp_options* opts, snp_system** out) 
             s->quad_lists = cluster_plan(s, T, &cp);
         }
     }
+    // no cluster holds it (wide emissions, or more than 65,408 neurons): in a
+    // batch one CTA does, where its packed emissions fit
+    if (s->has_grid && !s->quad_lists)
+        want_in = want_in && resident_smem_bytes(hp.q, resident_e_bits(hp.max_p)) + 1024 <= (size_t)optin;
     if (s->quad_lists)
         pack_in_quads(desc, &hp);
-    else if (want_in && !s->has_grid)
+    else if (want_in)
         pack_in_lists(desc, &hp);
-    s->has_in_lists = want_in && !s->quad_lists && !s->has_grid;
+    s->has_in_lists = want_in && !s->quad_lists;
     for (int lt = 0; lt < 4 && s->quad_lists; ++lt) {  // group i goes to CTA i mod T of a cluster
         std::vector<int32_t> cols((size_t)1 << lt, 0), rules((size_t)1 << lt, 0);
         for (size_t i = 0; i + 1 < hp.quad_ptr.size(); ++i) {
