@@ -34,6 +34,7 @@
 #include <thread>
 #include <vector>
 
+#include "autotune.h"
 #include "kernels.h"
 #include "snp_internal.h"
 #include "system.h"
@@ -59,71 +60,6 @@ struct Ticket {
 constexpr int64_t kRoundSteps = 64;          // steps per round and system
 constexpr int kSideStreams = 3;
 constexpr int kMaxRest = 4;  // widths of packed emissions: launches of the packed kernel in a round
-
-// Online autotuner of the resident launches.  A candidate is how many groups
-// of 128 neurons one CTA may hold: a system of more takes a cluster of 2, 4 or
-// 8 CTAs (kernels_cluster.cu), so a small bound shortens the largest systems
-// and a large one spends fewer CTAs and barriers.  Launches are grouped by
-// (bits per emission, log2 of the largest system); for each group every
-// candidate is tried on one real round (the work is not wasted: results do
-// not depend on the candidate), then the fastest by measured synaptic updates
-// per second is used.  With SNP_AUTOTUNE_CACHE naming a file, choices are read
-// at batch creation and written back at destroy (candidates are numbered from
-// kFirst there: the numbers below belonged to an earlier set).
-struct Autotune {
-    static constexpr int kN = 3;
-    static constexpr int kFirst = 6;
-    static int groups_of(int c) { return 16 << c; }
-    struct Stat {
-        double work[kN] = {0, 0, 0};
-        double secs[kN] = {0, 0, 0};
-        double top = 0;  // work of the largest round measured
-    };
-    std::map<std::pair<int, int>, Stat> stats;
-    int pick(const std::pair<int, int>& key) {
-        Stat& st = stats[key];
-        for (int c = 0; c < kN; ++c)
-            if (st.secs[c] == 0.0) return c;
-        int best = 0;
-        for (int c = 1; c < kN; ++c)
-            if (st.work[c] / st.secs[c] > st.work[best] / st.secs[best]) best = c;
-        return best;
-    }
-    // A round of much less work than another says nothing about it (systems join
-    // piecemeal at first): only rounds of at least half the largest one's work
-    // count, and a round of twice the work starts the comparison anew.
-    void record_round(const std::pair<int, int>& key, int c, double work, double secs) {
-        Stat& st = stats[key];
-        if (work < 0.5 * st.top) return;
-        if (work > 2.0 * st.top && st.top > 0.0) st = Stat();
-        st.top = std::max(st.top, work);
-        record(key, c, work, secs);
-    }
-    void record(const std::pair<int, int>& key, int c, double work, double secs) {
-        Stat& st = stats[key];
-        st.work[c] += work;
-        st.secs[c] += secs > 1e-9 ? secs : 1e-9;
-    }
-    void load(const char* path) {
-        FILE* f = path ? fopen(path, "r") : nullptr;
-        if (!f) return;
-        int eb, lq, c;
-        double w, t;
-        while (fscanf(f, "%d %d %d %lf %lf", &eb, &lq, &c, &w, &t) == 5)
-            if (c >= kFirst && c < kFirst + kN) record({eb, lq}, c - kFirst, w, t);
-        fclose(f);
-    }
-    void save(const char* path) const {
-        FILE* f = path ? fopen(path, "w") : nullptr;
-        if (!f) return;
-        for (const auto& kv : stats)
-            for (int c = 0; c < kN; ++c)
-                if (kv.second.secs[c] > 0.0)
-                    fprintf(f, "%d %d %d %.6g %.6g\n", kv.first.first, kv.first.second, c + kFirst, kv.second.work[c],
-                            kv.second.secs[c]);
-        fclose(f);
-    }
-};
 
 }  // namespace snp
 
@@ -264,8 +200,7 @@ static int run_resident_group(snp_batch* b, std::vector<snp_system*>& sys, std::
     const int e_bits = resident_e_bits(max_p);
     int lq = 0;
     while ((1 << lq) < max_q) ++lq;
-    const std::pair<int, int> key{e_bits, lq};
-    const int cand = b->tune.pick(key);
+    const int cand = b->tune.pick(e_bits, lq, work);
     std::vector<LaunchClass> cls(n);
     for (size_t i = 0; i < n; ++i) cls[i] = class_of(sys[i], Autotune::groups_of(cand), b->threads);
     std::vector<size_t> order(n);
@@ -343,7 +278,7 @@ static int run_resident_group(snp_batch* b, std::vector<snp_system*>& sys, std::
         float ms = 0.f;
         if (cudaEventElapsedTime(&ms, b->ev0, b->ev1) == cudaSuccess) {
             dev_seconds += ms * 1e-3;
-            b->tune.record_round(key, cand, work, ms * 1e-3);
+            b->tune.record(e_bits, lq, cand, work, ms * 1e-3);
         }
     }
     bool overflow = false, bounds = false;
