@@ -329,24 +329,27 @@ __global__ void __launch_bounds__(kNaThreads, 1) k_na_run(const __grid_constant_
             if (a < 0 || a > b || (long long)b > s.nin) {
                 invalid = true;
             } else {
-                const bool staged = a >= e_lo && b <= e_hi;
-                const int32_t* const p = staged ? esm + (a - e_lo) : s.in_src + a;
                 // eight emissions in flight: an index out of range gives none.
-                // Counted from 0 without a sign: a list may end at INT32_MAX.
-                const uint32_t len = (uint32_t)(b - a);
-                for (uint32_t e = 0u; e < len; e += 8u) {
-                    uint32_t v[8];
+                // What is left is counted down: a list may end at INT32_MAX.
+                auto gather = [&](const int32_t* p) {
+                    for (int32_t left = b - a; left > 0; left -= 8, p += 8) {
+                        uint32_t v[8];
 #pragma unroll
-                    for (uint32_t u = 0; u < 8u; ++u) {
-                        const bool there = e + u < len;
-                        const int32_t x = there ? p[e + u] : 0;
-                        const bool in = x >= 0 && x < s.q;
-                        invalid |= !in;
-                        v[u] = there && in ? __ldcg(Ek + x) : 0u;
+                        for (int u = 0; u < 8; ++u) {
+                            const bool there = u < left;
+                            const int32_t x = there ? p[u] : 0;
+                            const bool in = x >= 0 && x < s.q;
+                            invalid |= !in;
+                            v[u] = there && in ? __ldcg(Ek + x) : 0u;
+                        }
+#pragma unroll
+                        for (int u = 0; u < 8; ++u) sum += (long long)v[u];
                     }
-#pragma unroll
-                    for (uint32_t u = 0; u < 8u; ++u) sum += (long long)v[u];
-                }
+                };
+                if (a >= e_lo && b <= e_hi)
+                    gather(esm + (a - e_lo));
+                else
+                    gather(s.in_src + a);
             }
             int32_t c = Csm[i];
             const uint32_t st = Ssm[i];
