@@ -626,7 +626,8 @@ bool build_rule_tables(const snp_desc* d, HostPack* hp) {
     const bool terms = d->rule_term_offsets != nullptr;
     std::vector<int32_t> off((size_t)q);
     std::vector<uint32_t> tab, app;
-    std::vector<std::vector<int32_t>> lists;
+    // of one neuron: the rules of each entry counted, then dealt to their places
+    std::vector<int32_t> first, last;
     for (int32_t s = 0; s < q; ++s) {
         const int32_t i = hp->perm[s];
         const int64_t r0 = d->rule_offsets[i], r1 = d->rule_offsets[i + 1], R = r1 - r0;
@@ -647,31 +648,45 @@ bool build_rule_tables(const snp_desc* d, HostPack* hp) {
             }
         }
         if (K + L > cap) return false;
-        lists.assign((size_t)(K + L), {});
-        int64_t total = 0;
-        for (int64_t r = r0; r < r1; ++r)
-            for (int64_t u = terms ? d->rule_term_offsets[r] : r, e = terms ? d->rule_term_offsets[r + 1] : r + 1; u < e;
-                 ++u) {
-                const int64_t k = terms ? d->term_k[u] : d->rule_k[u], j = terms ? d->term_j[u] : d->rule_j[u];
-                for (int64_t n = k; n < K + L; n += j > 0 ? j : K + L) {  // entries K.. stand for n = K + (n - K) mod L
-                    if (n < d->rule_c[r]) continue;
-                    std::vector<int32_t>& x = lists[(size_t)n];
-                    if (!x.empty() && x.back() == (int32_t)(r - r0)) continue;  // another term of the rule
-                    x.push_back((int32_t)(r - r0));
-                    if (++total > cap) return false;
+        // every (entry, rule) pair in rule order, once (a rule's terms may share entries)
+        auto pairs = [&](auto visit) {
+            last.assign((size_t)(K + L), -1);
+            for (int64_t r = r0; r < r1; ++r)
+                for (int64_t u = terms ? d->rule_term_offsets[r] : r, e = terms ? d->rule_term_offsets[r + 1] : r + 1;
+                     u < e; ++u) {
+                    const int64_t k = terms ? d->term_k[u] : d->rule_k[u], j = terms ? d->term_j[u] : d->rule_j[u];
+                    for (int64_t n = k; n < K + L; n += j > 0 ? j : K + L) {  // entries K.. stand for n = K + (n - K) mod L
+                        if (n < d->rule_c[r] || last[(size_t)n] == (int32_t)(r - r0)) continue;
+                        last[(size_t)n] = (int32_t)(r - r0);
+                        if (!visit(n, r)) return false;
+                    }
                 }
-            }
+            return true;
+        };
+        int64_t total = 0;
+        first.assign((size_t)(K + L), 0);
+        if (!pairs([&](int64_t n, int64_t) {
+                first[(size_t)n]++;
+                return ++total <= cap;
+            }))
+            return false;
         off[s] = (int32_t)tab.size();
         tab.push_back((uint32_t)K | ((uint32_t)L << 16));
-        for (const std::vector<int32_t>& x : lists) {
-            tab.push_back((uint32_t)(app.size() / 2));
-            for (int32_t l : x) {
-                const int64_t r = r0 + l;
-                app.push_back((uint32_t)d->rule_c[r] | ((uint32_t)l << 16));
-                app.push_back((uint32_t)d->rule_p[r] | ((uint32_t)d->rule_d[r] << 16));
-            }
+        size_t at = app.size() / 2;
+        for (int32_t& f : first) {
+            tab.push_back((uint32_t)at);
+            const size_t n = (size_t)f;
+            f = (int32_t)at;
+            at += n;
         }
-        tab.push_back((uint32_t)(app.size() / 2));
+        tab.push_back((uint32_t)at);
+        app.resize(2 * at);
+        pairs([&](int64_t n, int64_t r) {
+            const size_t x = 2 * (size_t)first[(size_t)n]++;
+            app[x] = (uint32_t)d->rule_c[r] | ((uint32_t)(r - r0) << 16);
+            app[x + 1] = (uint32_t)d->rule_p[r] | ((uint32_t)d->rule_d[r] << 16);
+            return true;
+        });
         if (tab.size() > (size_t)INT32_MAX / 2) return false;
     }
     hp->tab_p.resize((size_t)hp->m);
