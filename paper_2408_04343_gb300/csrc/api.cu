@@ -853,8 +853,7 @@ int snp_create(const snp_desc* desc, const snp_options* opts, snp_system** out) 
     if (hp.quads && !s->compiled && !(s->tables = build_rule_tables(desc, &hp)))
         s->test_recs = build_test_records(desc, &hp);
     if (want_tiled && hp.quads && (int64_t)hp.max_in * (int64_t)hp.max_p <= (int64_t)INT32_MAX) {
-        quad_list_starts(hp, 1, &hp.quad_ptr32);
-        s->has_grid = grid_plan(s, hp, sms);
+        s->has_grid = quad_list_starts(hp, 1, &hp.quad_ptr32) && grid_plan(s, hp, sms);
         if (s->has_grid) {
             pack_in_quads32(desc, &hp, s->grid.e_bits);
             want_in = hp.q <= kBatchResidentMaxQ;  // for batches

@@ -116,14 +116,18 @@ void pack_in_lists(const snp_desc* d, HostPack* hp) {
     }
 }
 
-void quad_list_starts(const HostPack& hp, int per, std::vector<int32_t>* ptr) {
+bool quad_list_starts(const HostPack& hp, int per, std::vector<int32_t>* ptr) {
     const int32_t ng = (hp.q + kGroup - 1) / kGroup;
     ptr->assign((size_t)ng + 1, 0);
+    int64_t at = 0;
     for (int32_t g = 0; g < ng; ++g) {
         int32_t w = 0;
         for (int32_t s = g * kGroup; s < std::min(hp.q, (g + 1) * kGroup); ++s) w = std::max(w, hp.indeg[(size_t)hp.perm[s]]);
-        (*ptr)[g + 1] = (*ptr)[g] + (w + per - 1) / per;
+        at += ((int64_t)w + per - 1) / per;
+        if (at > INT32_MAX) return false;
+        (*ptr)[g + 1] = (int32_t)at;
     }
+    return true;
 }
 
 int32_t grid_longest_walk(const std::vector<int32_t>& ptr, int G, int warps, int warps_per_group) {
@@ -160,12 +164,12 @@ static void quad_columns(const snp_desc* d, const HostPack* hp, int per, std::ve
                 if (s >= 0) place[(size_t)hp->perm[s]] = g * kGroup + 4 * l + j;
             }
     const size_t np = (size_t)ng * kGroup;
-    std::vector<int32_t> off(np + 1, 0);
+    std::vector<int64_t> off(np + 1, 0);
     for (int32_t i = 0; i < q; ++i) off[(size_t)place[(size_t)i] + 1] = hp->indeg[(size_t)i];
     for (size_t x = 0; x < np; ++x) off[x + 1] += off[x];
     std::vector<int32_t> src((size_t)hp->nsyn);
     {
-        std::vector<int32_t> fill(off.begin(), off.end() - 1);
+        std::vector<int64_t> fill(off.begin(), off.end() - 1);
         for (int32_t i = 0; i < q; ++i)
             for (int64_t e = d->syn_offsets[i]; e < d->syn_offsets[i + 1]; ++e)
                 src[(size_t)fill[(size_t)place[(size_t)d->syn_targets[e]]]++] = place[(size_t)i];
@@ -184,14 +188,14 @@ static void quad_columns(const snp_desc* d, const HostPack* hp, int per, std::ve
     for (int32_t g = 0; g < ng; ++g) {
         const int32_t w = ((*ptr)[g + 1] - (*ptr)[g]) * per;
         const int32_t* const list = src.data() + off[(size_t)g * kGroup];
-        const int32_t* const at = off.data() + (size_t)g * kGroup;
-        if ((int32_t)next.size() < at[kGroup] - at[0]) next.resize((size_t)(at[kGroup] - at[0]));
+        const int64_t* const at = off.data() + (size_t)g * kGroup;
+        if ((int64_t)next.size() < at[kGroup] - at[0]) next.resize((size_t)(at[kGroup] - at[0]));
         for (int32_t x = 0; x < kGroup; ++x) {
             Banks& k = banks[(size_t)x];
             k.any = 0u;
             if (at[x] == at[x + 1]) continue;
             std::fill(k.head, k.head + 32, -1);
-            for (int32_t u = at[x] - at[0]; u < at[x + 1] - at[0]; ++u) {
+            for (int32_t u = (int32_t)(at[x] - at[0]); u < (int32_t)(at[x + 1] - at[0]); ++u) {
                 const int32_t b = word(list[u]) & 31;
                 next[(size_t)u] = k.head[b];
                 k.head[b] = u;

@@ -313,8 +313,9 @@ void pack_in_quads(const snp_desc* d, HostPack* hp);
 // one source of each of a lane's neurons per column, (byte address of the
 // source's word in the packed vector) << 8 | its first bit in the word.
 void pack_in_quads32(const snp_desc* d, HostPack* hp, int eb);
-// First columns of the groups' in-lists at `per` sources of each neuron per column.
-void quad_list_starts(const HostPack& hp, int per, std::vector<int32_t>* ptr);
+// First columns of the groups' in-lists at `per` sources of each neuron per
+// column; false when they do not fit 32 bits (never with 16-bit sources).
+bool quad_list_starts(const HostPack& hp, int per, std::vector<int32_t>* ptr);
 // Most columns one warp of the grid-resident engine walks: G CTAs of `warps`
 // warps, group g on CTA g mod G, there on one warp in turn or split over
 // warps_per_group of them.

@@ -36,6 +36,14 @@ int main() {
     bad += ptr != std::vector<int32_t>({0, 2, 79, 81});
     quad_list_starts(hp, 2, &ptr);
     bad += ptr != std::vector<int32_t>({0, 1, 40, 41});
+    // more columns than 32 bits count: 5,000 groups with a list of 600,000 each
+    hp.q = 5000 * kGroup;
+    hp.perm.resize((size_t)hp.q);
+    hp.indeg.assign((size_t)hp.q, 0);
+    for (int32_t i = 0; i < hp.q; ++i) hp.perm[(size_t)i] = i;
+    for (int32_t g = 0; g < 5000; ++g) hp.indeg[(size_t)g * kGroup + 5] = 600'000;
+    bad += quad_list_starts(hp, 1, &ptr);
+    bad += !quad_list_starts(hp, 2, &ptr) || ptr.back() != 5000 * 300'000;
     std::printf("bad=%d\n", bad);
     return bad;
 }
