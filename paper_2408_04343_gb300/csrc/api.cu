@@ -174,7 +174,8 @@ void build_plan(snp_system* s, std::vector<Piece>& plan) {
         }
         e.inflow = nullptr;
         if (s->opt.form == SNP_FORM_DENSE || inflow) fill(&e.inflow, q * 4, 0);
-        for (int b = 0; b < 2; ++b) fill(&e.Em[b], (size_t)hp.m + 1, 0);
+        e.Em[0] = e.Em[1] = nullptr;  // one-word pairs step on bits instead
+        for (int b = 0; b < 2 && im.ep.bit_ent.empty(); ++b) fill(&e.Em[b], (size_t)hp.m + 1, 0);
     }
     if (s->has_tiled) {
         TiledSys& tl = s->tiled;

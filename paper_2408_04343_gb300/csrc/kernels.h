@@ -137,7 +137,7 @@ struct EllSys {
     const int2* in_ent;      // (rule, p) pairs, pad (m, 0)
     const int32_t* out_ptr;  // out-ELL rule-slice starts (units of 32 pairs)
     const int2* out_ent;     // (target, p) pairs, pad (-1, 0)
-    uint8_t* Em[2];          // [m+1] rule r emits at step k: Em[k & 1][r]
+    uint8_t* Em[2];          // [m+1] rule r emits at step k: Em[k & 1][r] (NULL with bit_ent)
     // in-ELL in one word per pair (EllPack::bit_ent), or NULL
     const int32_t* bit_ptr;
     const uint4* bit_ent;
