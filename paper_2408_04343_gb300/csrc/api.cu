@@ -435,8 +435,8 @@ int effective_engine(const snp_system* s) {
 }
 
 static int step_grid(snp_system* s, int64_t n) {
-    for (int64_t done = 0; done < n; done += kGridMaxSteps)
-        if (launch_grid(s->dev, s->grid, std::min<int64_t>(n - done, kGridMaxSteps), done > 0, s->opt.select, s->stream) !=
+    for (int64_t done = 0; done < n; done += kLaunchMaxSteps)
+        if (launch_grid(s->dev, s->grid, std::min<int64_t>(n - done, kLaunchMaxSteps), done > 0, s->opt.select, s->stream) !=
             cudaSuccess)
             return cuda_fail("grid-resident launch");
     return SNP_OK;
@@ -536,8 +536,8 @@ static int step_ell_forms(snp_system* s, int64_t n) {
     cudaStream_t st = s->stream;
     const EllSys& e = s->ell;
     if (e.bit_ent) {
-        for (int64_t done = 0; done < n; done += kGridMaxSteps)
-            if (launch_ell_run(s->dev, e, std::min<int64_t>(n - done, kGridMaxSteps), done > 0, sel, st) != cudaSuccess)
+        for (int64_t done = 0; done < n; done += kLaunchMaxSteps)
+            if (launch_ell_run(s->dev, e, std::min<int64_t>(n - done, kLaunchMaxSteps), done > 0, sel, st) != cudaSuccess)
                 return cuda_fail("ell launch");
         return SNP_OK;
     }

@@ -90,8 +90,7 @@ struct GridSys {
     int32_t rules;             // as ClusterPlan::rules
 };
 size_t grid_smem_bytes(int mode, const GridSys& gs, bool lsm, int lsm_cols, int rules);
-// n <= kGridMaxSteps; more: a further launch of the same call.
-constexpr long long kGridMaxSteps = 1ll << 24;  // the barrier counters are 32 bits wide
+// n <= kLaunchMaxSteps; more: a further launch of the same call.
 cudaError_t launch_grid(const DevSys& s, const GridSys& gs, long long n, bool more, int sel, cudaStream_t st);
 // One forced step of nb configurations of one system (computation-tree
 // exploration); see k_branch_step.
@@ -152,7 +151,7 @@ struct EllSys {
 };
 cudaError_t launch_ell_pull(const DevSys& s, const EllSys& e, int kind, int32_t t, cudaStream_t st, bool compact,
                             int sel);
-// All steps of a call in one cooperative launch (bit_ent set); n <= kGridMaxSteps,
+// All steps of a call in one cooperative launch (bit_ent set); n <= kLaunchMaxSteps,
 // more as in launch_grid.
 cudaError_t launch_ell_run(const DevSys& s, const EllSys& e, long long n, bool more, int sel, cudaStream_t st);
 size_t ell_run_smem(const EllSys& e);

@@ -222,7 +222,6 @@ __device__ __forceinline__ SelOut na_select(const NaSys& s, const NaRules& rs, i
 }
 
 constexpr int kNaThreads = 512;
-constexpr int64_t kNaMaxSteps = 1ll << 24;  // of one launch: the barrier counters are 32 bits wide
 
 // Runs up to n steps from the base step.  Shared memory (smem bytes), for the
 // CTA's N neurons: spikes, status words, first rules, list starts, the rules
@@ -548,7 +547,7 @@ static cudaError_t na_run(const NaSys& s, const NaPlan& pl, int cap, int select,
     auto fn = select == SNP_SELECT_FIRST ? k_na_run<SNP_SELECT_FIRST> : k_na_run<SNP_SELECT_PHILOX>;
     // the same bound for every launch: threads may launch different sizes at once
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, cap - 1024);
-    for (int64_t done = 0; done < n && e == cudaSuccess; done += kNaMaxSteps) {
+    for (int64_t done = 0; done < n && e == cudaSuccess; done += kLaunchMaxSteps) {
         k_na_begin<<<1, 32, 0, st>>>(s, (unsigned long long)step, done == 0 ? 1 : 0);
         if ((e = cudaGetLastError()) != cudaSuccess) break;
         cudaLaunchConfig_t cfg = {};
@@ -561,7 +560,7 @@ static cudaError_t na_run(const NaSys& s, const NaPlan& pl, int cap, int select,
         at[0].val.cooperative = 1;
         cfg.attrs = at;
         cfg.numAttrs = 1;
-        e = cudaLaunchKernelEx(&cfg, fn, s, (long long)std::min<int64_t>(n - done, kNaMaxSteps), pl.N, pl.smem,
+        e = cudaLaunchKernelEx(&cfg, fn, s, (long long)std::min<int64_t>(n - done, kLaunchMaxSteps), pl.N, pl.smem,
                                done > 0 ? 1 : 0);
     }
     return e;

@@ -16,6 +16,15 @@
 
 namespace snp {
 
+// Most steps of one cooperative launch: the counters its CTAs meet at are 32 bits
+// wide.  The bounds-checked build takes few, so that its tests reach the
+// launches that continue a call.
+#ifdef SNP_CHECK_BOUNDS
+constexpr int64_t kLaunchMaxSteps = 7;
+#else
+constexpr int64_t kLaunchMaxSteps = 1ll << 24;
+#endif
+
 // Neurons are processed in slices of 32 (one warp, one neuron per lane).
 constexpr int kSlice = 32;
 // Status word of a neuron: low 16 bits = D (steps until it reopens), high
