@@ -91,8 +91,11 @@ extern "C" {
  *                          into shared memory (in source partitions when it
  *                          does not fit at once) so in-neighbour reads are
  *                          shared-memory reads; the default for large
- *                          systems under AUTO, where middle-sized ones run
- *                          all steps of a call in one cooperative launch.   */
+ *                          systems under AUTO, where middle-sized ones
+ *                          without long in-lists run all steps of a call in
+ *                          one cooperative launch, as the ELL form's pull
+ *                          does: it starts when all its CTAs (up to one per
+ *                          SM) fit beside what runs on other streams.       */
 #define SNP_ENGINE_TILED 3
 
 /* Optional device allocator (e.g. a framework's caching allocator).  Both

@@ -9,7 +9,9 @@
 //  2. one round -- every admitted system advances by up to `round` steps.
 //     Systems of up to 65,408 neurons run on the cluster-resident engine, a
 //     cluster of 1 to 8 CTAs per system, in one launch per cluster size and
-//     kernel instance over a table of system descriptors, the largest first.  Larger systems run on the grid-wide engines on
+//     kernel instance over a table of system descriptors, the largest first;
+//     what fits no cluster, up to 65,536 neurons, takes a CTA each with packed
+//     emissions.  Larger systems run on the grid-wide engines on
 //     their own streams at the same time, so their work overlaps;
 //  3. retirement -- systems that used up their steps or reached a fixed
 //     point leave; a ticket completes when all its systems have.

@@ -18,7 +18,8 @@
 // The launch is cooperative, so all CTAs are resident; the wait is bounded all
 // the same.  us per step, a launch per step / so: 9,000 neurons 8.1 / 3.0,
 // 32,768 8.2 / 3.3, 100,003 9.1 / 4.0, 200,003 9.9 / 5.7, 450,000 12.8 / 9.4;
-// 100,003 neurons of wide rules 17.6 / 6.0.
+// 100,003 neurons of wide rules 17.6 / 6.0.  Systems with long in-lists are left
+// to the tiled engine (grid_plan in api.cu says where the line lies).
 #include <cuda_runtime.h>
 
 #include <algorithm>
