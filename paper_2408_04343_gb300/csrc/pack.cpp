@@ -924,7 +924,12 @@ int pack_tiled(const snp_desc* d, const HostPack& hp, int G, size_t smem_budget,
         std::vector<int64_t> gstart;                       // first entry of each target group
         std::vector<std::vector<std::pair<uint32_t, int64_t>>> tmpl(T);  // per run: (advance, seq index or -1)
         const uint32_t dummy = (uint32_t)max_slots;       // the accumulator no slot reads
-        for (int g = 0; g < NR; ++g) {
+        // short runs spend most of their words on padding: the run-length layout
+        // is kept only when it is clearly smaller, and one long run per CTA
+        // (every run of a CTA is as long as its longest) can settle that
+        const double most_words = tp->acc8 ? 1e300 : 0.9 * other_words;
+        bool smaller = true;
+        for (int g = 0; g < NR && smaller; ++g) {
             for (int h = 0; h < P; ++h) {
                 const int c = g * P + h;
                 int32_t* sb = tp->sub.data() + (size_t)c * (kTiledMaxSub + 1);
@@ -987,6 +992,10 @@ int pack_tiled(const snp_desc* d, const HostPack& hp, int G, size_t smem_budget,
                         hi_c = mid;
                     else
                         lo_c = mid + 1;
+                }
+                if ((double)tp->ent.size() + (double)((lo_c + 4) / 5 * T * 4) > most_words) {
+                    smaller = false;
+                    break;
                 }
                 fits(lo_c, true);
                 // the positions of every run: the advance of each entry and the
@@ -1085,9 +1094,7 @@ int pack_tiled(const snp_desc* d, const HostPack& hp, int G, size_t smem_budget,
                 if (tp->ent.size() > (size_t)INT32_MAX) return fail(SNP_ERR_UNSUPPORTED, "too many entries");
             }
         }
-        // short runs spend most of their words on padding: keep the run-length
-        // layout only when it is clearly smaller
-        if (tp->acc8 || (double)tp->ent.size() <= 0.9 * other_words) {
+        if (smaller && (double)tp->ent.size() <= most_words) {
             tp->pairs = 0;
             // slack: the gather loads two vectors ahead of the one it adds,
             // so the last CTA's threads read up to two rows past its block
