@@ -203,6 +203,24 @@ void build_plan(snp_system* s, std::vector<Piece>& plan) {
     }
 }
 
+// Id of the current context, unique for the life of the process (0: unknown):
+// after cudaDeviceReset the same device has another one.
+static unsigned long long context_id() {
+    using Fn = CUresult (*)(CUcontext, unsigned long long*);
+    static const Fn fn = [] {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &p, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            p = nullptr;
+        }
+        return reinterpret_cast<Fn>(p);
+    }();
+    unsigned long long id = 0;
+    return fn && fn(nullptr, &id) == CUDA_SUCCESS ? id : 0;
+}
+
 int materialize(snp_system* s) {
     if (s->materialized) return SNP_OK;
     if (!s->img) return fail(SNP_ERR_INVALID, "system has no host image");
@@ -237,6 +255,7 @@ int materialize(snp_system* s) {
         return cuda_fail("descriptor upload");
     if (cudaStreamSynchronize(s->stream) != cudaSuccess) return cuda_fail("upload sync");
     s->img.reset();
+    s->context = context_id();
     s->materialized = true;
     return SNP_OK;
 }
@@ -569,24 +588,6 @@ static int step_ell_forms(snp_system* s, int64_t n) {
     return SNP_OK;
 }
 
-// Id of the current context, unique for the life of the process (0: unknown):
-// after cudaDeviceReset the same device has another one.
-static unsigned long long context_id() {
-    using Fn = CUresult (*)(CUcontext, unsigned long long*);
-    static const Fn fn = [] {
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &p, 12000, cudaEnableDefault, &q) != cudaSuccess ||
-            q != cudaDriverEntryPointSuccess) {
-            cudaGetLastError();
-            p = nullptr;
-        }
-        return reinterpret_cast<Fn>(p);
-    }();
-    unsigned long long id = 0;
-    return fn && fn(nullptr, &id) == CUDA_SUCCESS ? id : 0;
-}
-
 // Page-locked bytes for small reads back, one piece per thread and context for
 // as long as both live: a copy into pageable memory is staged by the driver,
 // about 5 us each time (a piece per system would cost its creation 100 us and
@@ -609,13 +610,14 @@ struct PinnedWords {
             }
     }
 };
-static void* pinned_words() {
+// id: of the context whose memory is read.
+static void* pinned_words(unsigned long long id) {
     static thread_local PinnedWords w;
-    const unsigned long long id = context_id();
     if (id == 0) return nullptr;
     for (int i = 0; i < PinnedWords::kContexts; ++i) {
         if (w.ctx[i] == id) return w.p[i];
         if (w.ctx[i] != 0) continue;
+        if (context_id() != id) return nullptr;  // another context is current: not its own bytes
         w.ctx[i] = id;  // asked for once, whatever comes of it
         if (cudaHostAlloc(&w.p[i], kStatusBytes, cudaHostAllocDefault) != cudaSuccess) {
             cudaGetLastError();
@@ -626,11 +628,11 @@ static void* pinned_words() {
     return nullptr;
 }
 
-// Copies `bytes` (at most kStatusBytes) from the device and waits.
-static bool read_small(void* dst, const void* src, size_t bytes, cudaStream_t st) {
-    void* pin = pinned_words();
-    if (cudaMemcpyAsync(pin ? pin : dst, src, bytes, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaStreamSynchronize(st) != cudaSuccess)
+// Copies `bytes` (at most kStatusBytes) from the system's device memory and waits.
+static bool read_small(const snp_system* s, void* dst, const void* src, size_t bytes) {
+    void* pin = pinned_words(s->context);
+    if (cudaMemcpyAsync(pin ? pin : dst, src, bytes, cudaMemcpyDeviceToHost, s->stream) != cudaSuccess ||
+        cudaStreamSynchronize(s->stream) != cudaSuccess)
         return false;
     if (pin) std::memcpy(dst, pin, bytes);
     return true;
@@ -638,7 +640,7 @@ static bool read_small(void* dst, const void* src, size_t bytes, cudaStream_t st
 
 int read_flags(snp_system* s, int64_t* exec) {
     alignas(8) unsigned char words[kStatusBytes];
-    if (!read_small(words, s->dev.flags, kStatusBytes, s->stream)) return cuda_fail("flag read");
+    if (!read_small(s, words, s->dev.flags, kStatusBytes)) return cuda_fail("flag read");
     uint32_t fl[kNumFlags];
     unsigned long long steps[kNumStepWords];
     std::memcpy(fl, words, sizeof(fl));
@@ -1218,7 +1220,7 @@ int snp_get_state(const snp_system* s, int32_t* C, int32_t* D, int32_t* P, int64
     if (P && (rc = snp_get_pending(s, P, len))) return rc;
     if (step) {
         unsigned long long v = 0;
-        if (!read_small(&v, s->dev.step + kStepBase, sizeof(v), s->stream))
+        if (!read_small(s, &v, s->dev.step + kStepBase, sizeof(v)))
             return cuda_fail("step read");
         *step = v;
     }
@@ -1259,7 +1261,7 @@ int snp_set_state(snp_system* s, const int32_t* C, const int32_t* D, const int32
     if (!direct && (cudaMemsetAsync(s->dev.S[0], 0xff, bytes, st) != cudaSuccess ||
                     cudaMemsetAsync(s->dev.S[1], 0xff, bytes, st) != cudaSuccess))
         return cuda_fail("state upload");
-    if (!read_small(&bad, s->dev.flags + kFlagImport, sizeof(bad), st)) return cuda_fail("state import");
+    if (!read_small(s, &bad, s->dev.flags + kFlagImport, sizeof(bad))) return cuda_fail("state import");
     if (bad != 0xffffffffu) {
         if (direct && (cudaMemsetAsync(s->dev.S[0], 0xff, bytes, st) != cudaSuccess ||
                        cudaMemsetAsync(s->dev.S[1], 0xff, bytes, st) != cudaSuccess ||

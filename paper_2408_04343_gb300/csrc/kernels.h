@@ -26,8 +26,8 @@ cudaError_t launch_export(const DevSys& s, const int32_t* rule_base, int what, i
 // range in flags[kFlagImport] (which the caller sets to 0xffffffff first); the
 // commit, if there is none, writes C and the status words in slot order, the
 // step words and flags.  hold (q words): C, D and P are the caller's arrays; what
-// the check read of them is kept there and in the spiking vectors, and is what
-// the commit writes.  NULL: they are private copies, read by both launches.
+// the check read of them is kept there and in a spiking vector, and is what the
+// commit writes; the spiking vectors are left at -1.  NULL: they are private copies, read by both launches.
 cudaError_t launch_import(const DevSys& s, const int32_t* rule_base, const int32_t* C, const int32_t* D,
                           const int32_t* P, unsigned long long step, int32_t* hold, cudaStream_t st);
 

@@ -298,9 +298,11 @@ __global__ void k_export(const DevSys s, const int32_t* __restrict__ rule_base, 
 // flags.  Both launches go out at once: the second reads the first one's
 // verdict, so the host waits once.
 // hold: C, D and P are the caller's own arrays, which another stream may still
-// write.  Each value is then read once: the check keeps what it read, in slot
-// order, in hold and the spiking vectors; the commit writes that and leaves the
-// spiking vectors at -1.
+// write.  Each value is then read once: the check keeps the spikes and the
+// status words it made of what it read, in slot order, in hold and a spiking
+// vector; the commit writes those (reading 8 bytes per neuron, not the three
+// arrays and the slot's neuron and rules again) and leaves the spiking vectors
+// at -1.
 template <bool COMMIT>
 __global__ void k_import(DevSys s, const int32_t* __restrict__ rule_base, const int32_t* __restrict__ C,
                          const int32_t* __restrict__ D, const int32_t* __restrict__ P, unsigned long long step,
@@ -318,30 +320,31 @@ __global__ void k_import(DevSys s, const int32_t* __restrict__ rule_base, const 
         }
     }
     if (slot >= s.q) return;
-    const uint32_t i = neuron_id(s, slot);
-    const bool held = COMMIT && hold != nullptr;
-    const int32_t c = held ? hold[slot] : *(const volatile int32_t*)(C + i);
-    const int32_t d = held ? s.S[0][slot] : *(const volatile int32_t*)(D + i);
-    const int32_t p = held ? s.S[1][slot] : *(const volatile int32_t*)(P + i);
-    const int32_t r0 = rule_base[slot];
-    if (!COMMIT) {
-        bool ok = c >= 0 && d >= 0 && d <= kMaxDelay;
-        if (p == -1)
-            ok = ok && d == 0;
-        else
-            ok = ok && p >= r0 && p - r0 < rule_hi(s, slot) - rule_lo(s, slot);
-        if (!ok) atomicMin(s.flags + kFlagImport, i);
-        if (hold) {
-            hold[slot] = c;
-            s.S[0][slot] = d;
-            s.S[1][slot] = p;
-        }
+    if (COMMIT && hold) {
+        s.C[slot] = hold[slot];
+        s.st[slot] = (uint32_t)s.S[0][slot];
+        s.S[0][slot] = -1;
         return;
     }
-    s.C[slot] = c;
-    s.st[slot] = p == -1 ? 0u : ((uint32_t)(p - r0 + 1) << kPendShift) | (uint32_t)d;
-    if (held) {
-        s.S[0][slot] = -1;
+    const uint32_t i = neuron_id(s, slot);
+    const int32_t c = *(const volatile int32_t*)(C + i), d = *(const volatile int32_t*)(D + i),
+                  p = *(const volatile int32_t*)(P + i);
+    const int32_t r0 = rule_base[slot];
+    const uint32_t st = p == -1 ? 0u : (((uint32_t)p - (uint32_t)r0 + 1u) << kPendShift) | (uint32_t)d;
+    if (COMMIT) {
+        s.C[slot] = c;
+        s.st[slot] = st;
+        return;
+    }
+    bool ok = c >= 0 && d >= 0 && d <= kMaxDelay;
+    if (p == -1)
+        ok = ok && d == 0;
+    else
+        ok = ok && p >= r0 && p - r0 < rule_hi(s, slot) - rule_lo(s, slot);
+    if (!ok) atomicMin(s.flags + kFlagImport, i);
+    if (hold) {
+        hold[slot] = c;
+        s.S[0][slot] = (int32_t)st;
         s.S[1][slot] = -1;
     }
 }

@@ -91,6 +91,7 @@ struct snp_system {
     // deferred upload
     std::unique_ptr<snp::HostImage> img;  // host layouts until uploaded
     bool materialized = false;
+    unsigned long long context = 0;  // id of the context that holds its memory (0: unknown)
     size_t planned_bytes = 0;             // device bytes the upload will take
     struct snp_batch* owner = nullptr;    // batch that uploaded it (memory accounting)
     bool own_stream = false;              // stream created by the library
